@@ -95,10 +95,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) cg_cluster_kernel(const MdagmA
       int i = 0, j = 0, c = 0;
       bond_of(a.g, f + 1, ok ? b : 0, i, j, c);
       u[f] = ok ? __ldg(a.U + 2 * ((size_t)(tb + sl) * V + i) + c) : make_double2(0.0, 0.0);
-      if (FX) {
-        const long long re = __double2ll_rn(u[f].x * 0x1p64), im = __double2ll_rn(u[f].y * 0x1p64);
-        uf[f] = make_int4(fx_hi(re), fx_lo(re), fx_hi(im), fx_lo(im));
-      }
+      if (FX) uf[f] = fx_link_limbs(__double2ll_rn(u[f].x * 0x1p64), __double2ll_rn(u[f].y * 0x1p64));
       ij[f] = ok ? (sl * V + i) | ((sl * V + j) << 16) : -1;
     }
   }

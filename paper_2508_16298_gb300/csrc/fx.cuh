@@ -179,6 +179,15 @@ HQMC_HD int fx_link_index(int L, int x, int y, int c) {
   return 2 * L * Lh + (((y & 1) * Lh + (y >> 1)) * 2 + (x & 1)) * Lh + (x >> 1);
 }
 
+// Limbs of the link (re, im), in units of 2^-64.  conj(u) and -u are formed limb by limb,
+// and a low limb of -2^31 has no negative in 32 bits: such a component moves by one unit
+// (left as it is, one link in 2^31 had cross terms of the wrong sign, 2^-32 of the product).
+HQMC_HD int4 fx_link_limbs(long long re, long long im) {
+  re += fx_lo(re) == INT32_MIN ? 1 : 0;
+  im += fx_lo(im) == INT32_MIN ? 1 : 0;
+  return make_int4(fx_hi(re), fx_lo(re), fx_hi(im), fx_lo(im));
+}
+
 HQMC_HD double fx_link_part(int h, int l) { return (double)h * 0x1p-32 + (double)l * 0x1p-64; }
 HQMC_HD double2 fx_link_to_double(int4 u) {
   if (u.x == kFxBadLink) {

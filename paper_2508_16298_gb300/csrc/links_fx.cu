@@ -58,9 +58,9 @@ __device__ __forceinline__ FxLink fx_link(double theta, const longlong2* __restr
   return FxLink{make_longlong2(0, 0), false};
 }
 
-__device__ __forceinline__ int4 fx_link_limbs(const FxLink& k) {
+__device__ __forceinline__ int4 fx_limbs(const FxLink& k) {
   if (!k.finite) return make_int4(kFxBadLink, 0, 0, 0);
-  return make_int4(fx_hi(k.u.x), fx_lo(k.u.x), fx_hi(k.u.y), fx_lo(k.u.y));
+  return fx_link_limbs(k.u.x, k.u.y);
 }
 __device__ __forceinline__ float2 fx_link_float(const FxLink& k) {
   if (!k.finite) return make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000));
@@ -89,8 +89,8 @@ __device__ __forceinline__ void links_fx_part(const Geo& g, const double* __rest
       const FxLink uy = fx_link(th.y, tab + 256, t2);
       if (o.UF) {
         const int x = s % g.L, y = s / g.L;
-        o.UF[2 * base + fx_link_index(g.L, x, y, 0)] = fx_link_limbs(ux);
-        o.UF[2 * base + fx_link_index(g.L, x, y, 1)] = fx_link_limbs(uy);
+        o.UF[2 * base + fx_link_index(g.L, x, y, 0)] = fx_limbs(ux);
+        o.UF[2 * base + fx_link_index(g.L, x, y, 1)] = fx_limbs(uy);
         bad |= !ux.finite || !uy.finite;
       }
       if (o.U32) {

@@ -129,3 +129,55 @@ def test_gauss_pairs(lib):
             w = 2 * mpmath.pi * mpmath.mpf(int(bi)) / 2 ** 53
             for v, e in ((x, r * mpmath.cos(w)), (y, r * mpmath.sin(w))):
                 assert abs(mpmath.mpf(float(v)) - e) < 2.0 ** -56 * max(1, r) + 2.0 ** -53 * abs(e), (int(ai), int(bi))
+
+
+PRODUCTS = r"""
+#include "fx.cuh"
+using namespace hqmc;
+extern "C" {
+// u b and conj(u) b, then (-u) b and conj(-u) b as the force's step back forms them
+void products(const long long* u, const long long* b, long long* o, int n) {
+  for (int i = 0; i < n; ++i) {
+    const longlong2 z = make_longlong2(0, 0), x = make_longlong2(b[2 * i], b[2 * i + 1]);
+    const int4 k = fx_link_limbs(u[2 * i], u[2 * i + 1]), m = make_int4(-k.x, -k.y, -k.z, -k.w);
+    const longlong2 r[4] = {cfma(z, k, x), cfmac(z, k, x), cfma(z, m, x), cfmac(z, m, x)};
+    for (int j = 0; j < 4; ++j) { o[8 * i + 2 * j] = r[j].x; o[8 * i + 2 * j + 1] = r[j].y; }
+  }
+}
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def products_lib(tmp_path_factory):
+    return compile_host(tmp_path_factory, PRODUCTS)
+
+
+def compile_host(tmp_path_factory, text):
+    if not os.path.exists(NVCC):
+        pytest.skip("nvcc not found")
+    d = tmp_path_factory.mktemp("fx")
+    src, so = str(d / "fx.cu"), str(d / "fx.so")
+    open(src, "w").write(text)
+    subprocess.check_call([NVCC, "-gencode", "arch=compute_103a,code=sm_103a", "-O2", "-std=c++17", "-shared", "-Xcompiler", "-fPIC",
+                           "-I" + CSRC, src, "-o", so])
+    return ctypes.CDLL(so)
+
+
+def test_link_products_at_the_ends_of_the_low_limb(products_lib):
+    """A link's low limb at -2^31, next to it and at 2^31 - 1: u b, conj(u) b and their
+    negatives against exact integers.  A product is within 2 units: 1/2 of rounding, 1/4 for
+    each product of two low limbs, and |b| 2^-64 < 1/2 for each component moved by a unit."""
+    lows = [-2 ** 31, -2 ** 31 + 1, -1, 0, 1, 2 ** 31 - 1]
+    highs = [0x1199999A, -0x0CCCCCCD, 0x4CCCCCCC, 0]
+    b = [(2 ** 58 + 12345, -2 ** 59 + 2 ** 31), (-3 * 2 ** 57, 2 ** 60 - 1), (2 ** 31, -2 ** 31)]
+    cases = [(h * 2 ** 32 + lo, h2 * 2 ** 32 + l2, x, y) for h in highs for lo in lows for h2 in highs[:2] for l2 in lows
+             for x, y in b]
+    u = np.array([c[:2] for c in cases], dtype=np.int64)
+    v = np.array([c[2:] for c in cases], dtype=np.int64)
+    o = np.empty((len(cases), 4, 2), np.int64)
+    products_lib.products(ptr(u), ptr(v), ptr(o), len(cases))
+    for (ur, ui, x, y), r in zip(cases, o):
+        for (sr, si), (pr, pi) in zip(((1, 1), (1, -1), (-1, -1), (-1, 1)), r):
+            er, ei = sr * ur * x - si * ui * y, sr * ur * y + si * ui * x
+            assert abs(Fraction(er, 2 ** 64) - int(pr)) <= 2 and abs(Fraction(ei, 2 ** 64) - int(pi)) <= 2, (ur, ui, x, y)
