@@ -50,17 +50,6 @@ FxForceScales fx_force_scales(double a) {
   return s;
 }
 
-// (d.x u.y - d.y u.x) 2^(shift - 64), rounded.
-__device__ __forceinline__ long long fx_im(longlong2 d, longlong2 u, int shift) {
-  const int dxh = fx_hi(d.x), dxl = fx_lo(d.x), dyh = -fx_hi(d.y), dyl = -fx_lo(d.y);
-  const int uxh = fx_hi(u.x), uxl = fx_lo(u.x), uyh = fx_hi(u.y), uyl = fx_lo(u.y);
-  const long long hh = fx_madw(dyh, uxh, fx_madw(dxh, uyh, 0));
-  // the cross terms and the high words of the low limbs' products, with half a unit of the result
-  const long long low = (long long)__mulhi(dxl, uyl) + __mulhi(dyl, uxl) + (1ll << (31 - shift));
-  const long long c = fx_madw(dyl, uxh, fx_madw(dyh, uxl, fx_madw(dxl, uyh, fx_madw(dxh, uyl, low))));
-  return (hh << shift) + (c >> (32 - shift));
-}
-
 // (vi, vj) <- (1 - U T)(vi, vj)
 __device__ __forceinline__ void bond2_back(longlong2& vi, longlong2& vj, const int4 u) {
   bond2(vi, vj, make_int4(-u.x, -u.y, -u.z, -u.w));

@@ -289,8 +289,28 @@ HQMC_HD long long fx_mulhi(long long a, long long b) {
   return (long long)(((__int128)a * b) >> 64);
 #endif
 }
+HQMC_HD int fx_mulhi32(int a, int b) {
+#if defined(__CUDA_ARCH__)
+  return __mulhi(a, b);
+#else
+  return (int)(((long long)a * b) >> 32);
+#endif
+}
 HQMC_HD unsigned fx_umulhi32(unsigned a, unsigned b) {
   return (unsigned)(((unsigned long long)a * b) >> 32);
+}
+
+// (d.x u.y - d.y u.x) 2^(shift - 64), rounded.  d.y is negated before it is split: its low
+// limb may be -2^31, which has no negative.
+HQMC_HD long long fx_im(longlong2 d, longlong2 u, int shift) {
+  const long long ny = -d.y;
+  const int dxh = fx_hi(d.x), dxl = fx_lo(d.x), dyh = fx_hi(ny), dyl = fx_lo(ny);
+  const int uxh = fx_hi(u.x), uxl = fx_lo(u.x), uyh = fx_hi(u.y), uyl = fx_lo(u.y);
+  const long long hh = fx_madw(dyh, uxh, fx_madw(dxh, uyh, 0));
+  // the cross terms and the high words of the low limbs' products, with half a unit of the result
+  const long long low = (long long)fx_mulhi32(dxl, uyl) + fx_mulhi32(dyl, uxl) + (1ll << (31 - shift));
+  const long long c = fx_madw(dyl, uxh, fx_madw(dyh, uxl, fx_madw(dxl, uyh, fx_madw(dxh, uyl, low))));
+  return (hh << shift) + (c >> (32 - shift));
 }
 
 // s (cos, sin) of f turns for a table of s (cos, sin)(2 pi k / 256), in the table's units.

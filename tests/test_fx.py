@@ -181,3 +181,30 @@ def test_link_products_at_the_ends_of_the_low_limb(products_lib):
         for (sr, si), (pr, pi) in zip(((1, 1), (1, -1), (-1, -1), (-1, 1)), r):
             er, ei = sr * ur * x - si * ui * y, sr * ur * y + si * ui * x
             assert abs(Fraction(er, 2 ** 64) - int(pr)) <= 2 and abs(Fraction(ei, 2 ** 64) - int(pi)) <= 2, (ur, ui, x, y)
+
+
+PRODUCT_SUMS = r"""
+#include "fx.cuh"
+extern "C" void im(const long long* d, const long long* u, int shift, long long* o, int n) {
+  for (int i = 0; i < n; ++i)
+    o[i] = hqmc::fx_im(make_longlong2(d[2 * i], d[2 * i + 1]), make_longlong2(u[2 * i], u[2 * i + 1]), shift);
+}
+"""
+
+
+def test_product_sums_at_the_ends_of_the_low_limb(tmp_path_factory):
+    """The force's d.x u.y - d.y u.x with low words 2^31, next to it and 2^31 - 1 in every
+    place, against exact integers.  In units of 2^(64 - shift): 1/2 of rounding and two
+    high words cut by up to 1 of 2^32 each, so within 1."""
+    lib = compile_host(tmp_path_factory, PRODUCT_SUMS)
+    lows = [2 ** 31, 2 ** 31 + 1, 2 ** 31 - 1, 0]
+    hi = [2 ** 24 + 1, -2 ** 25, 3, -1]
+    cases = [[(h * 2 ** 32 + x) for h, x in zip(hi[k:] + hi[:k], (a, b, c, d))]
+             for k in range(4) for a in lows for b in lows for c in lows for d in lows]
+    q = np.array(cases, dtype=np.int64)
+    d, u = np.ascontiguousarray(q[:, :2]), np.ascontiguousarray(q[:, 2:])
+    for shift in (4, 10):  # sums of high limbs below 2^51: no shift above 11 (fx_force_scales)
+        o = np.empty(len(q), np.int64)
+        lib.im(ptr(d), ptr(u), shift, ptr(o), len(q))
+        for (dx, dy, ux, uy), r in zip(cases, o):
+            assert abs(Fraction(dx * uy - dy * ux, 2 ** (64 - shift)) - int(r)) <= 1, (dx, dy, ux, uy)
