@@ -153,12 +153,14 @@ HQMC_HD double fx_to_double_normal(long long v, int e) {
   const unsigned long long bits = ((unsigned long long)(1085 - lz + e) << 52) + m;
   return fx_from_bits((long long)(bits | ((unsigned long long)sg & (1ull << 63))));
 }
-// The same for any e a slice can have (uniform over a block): far from the middle of
-// the exponent range the result is formed 2^512 away and scaled, so that it
-// underflows and overflows as FP64 does.
+// The same for any e (uniform over a block): far from the middle of the exponent range the
+// result is formed 2^512 away and scaled, so that it underflows and overflows as FP64
+// does.  The exponent of a product of two slices goes far beyond what one such step
+// covers (to -2160 and 2000); below 2^-1300 every v is zero, above 2^1100 infinite.
 HQMC_HD double fx_to_double(long long v, int e) {
   if (e > -800 && e < 800) return fx_to_double_normal(v, e);
-  return e < 0 ? fx_to_double_normal(v, e + 512) * 0x1p-512 : fx_to_double_normal(v, e - 512) * 0x1p512;
+  return e < 0 ? fx_to_double_normal(v, (e < -1300 ? -1300 : e) + 512) * 0x1p-512
+               : fx_to_double_normal(v, (e > 1100 ? 1100 : e) - 512) * 0x1p512;
 }
 
 // v 2^-n rounded, n >= 0 (uniform over a block).

@@ -208,3 +208,30 @@ def test_product_sums_at_the_ends_of_the_low_limb(tmp_path_factory):
         lib.im(ptr(d), ptr(u), shift, ptr(o), len(q))
         for (dx, dy, ux, uy), r in zip(cases, o):
             assert abs(Fraction(dx * uy - dy * ux, 2 ** (64 - shift)) - int(r)) <= 1, (dx, dy, ux, uy)
+
+
+TO_DOUBLE = r"""
+#include "fx.cuh"
+extern "C" void to_double_any(const long long* v, const int* e, double* o, int n) {
+  for (int i = 0; i < n; ++i) o[i] = hqmc::fx_to_double(v[i], e[i]);
+}
+"""
+
+
+def test_to_double_at_any_exponent(tmp_path_factory):
+    """v 2^e for the exponents of a slice and of a product of two slices: rounded as FP64 rounds
+    it where v has 53 bits (one rounding, subnormal results included), zero below the range
+    and infinite above it."""
+    lib = compile_host(tmp_path_factory, TO_DOUBLE)
+    g = np.random.default_rng(15)
+    vs = np.concatenate([g.integers(-2 ** 53, 2 ** 53, 20), [0, 1, -1, 12345, 2 ** 60, -(2 ** 62)]])
+    es = [-4300, -2400, -2100, -1800, -1700, -1600, -1500, -1301, -1300, -1200, -1138, -1137, -1100, -1074, -1000, -801, -800,
+          -799, -60, 0, 799, 800, 801, 960, 1000, 1023, 1024, 1100, 1101, 1500, 1600, 1934, 2100]
+    v = np.repeat(vs, len(es)).astype(np.int64)
+    e = np.tile(es, len(vs)).astype(np.int32)
+    o = np.empty(len(v))
+    lib.to_double_any(ptr(v), ptr(e), ptr(o), len(v))
+    with np.errstate(over="ignore", under="ignore"):
+        want = np.ldexp(v.astype(np.float64), e)
+    bad = ~(o == want)
+    assert not np.any(bad), list(zip(v[bad], e[bad], o[bad], want[bad]))[:5]

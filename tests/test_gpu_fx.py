@@ -277,3 +277,25 @@ def test_batch_kernels_of_smaller_lattices(hq, L, N):
             X, i = hq.cg_solve(cfg, cuda(th), cuda(x), tol=1e-9, solver=solver)
             res = x - oracle.apply_MdagM(lat, th, X.cpu().numpy())
             assert i["status"] == 0 and np.linalg.norm(res) <= 1.01e-9 * np.linalg.norm(x)
+
+
+@pytest.mark.parametrize("L", [18, 54])
+def test_force_at_the_ends_of_the_exponent_range(hq, L):
+    """dS_f is bilinear in X: below 1e-162 its terms underflow and above 1e154 they overflow, as
+    in FP64, also where a product of two slices' exponents is far outside a double's.  Mixed
+    slices: a tiny slice beside a huge one, whose products are of order one."""
+    N = 6
+    lat = oracle.Lattice(L, N)
+    th, base = inputs.theta_hot(L, N, seed=97), inputs.complex_gaussian(L, N, seed=98)
+    mixed = base.copy()
+    mixed[0::2] *= 1e-140
+    mixed[1::2] *= 1e140
+    with hq.Config(L, N) as cfg, np.errstate(all="ignore"):
+        for x in (base * 1e-250, base * 1e-230, base * 1e-200, base * 1e-160, base * 1e150, base * 1e200, base * 1e250, mixed):
+            d = torch.empty((N, L, L, 2), dtype=torch.float64, device="cuda")
+            hq.force(cfg, cuda(th), cuda(x), dSf=d)
+            d, do = d.cpu().numpy(), oracle.fermion_dS(lat, th, x)
+            assert np.array_equal(np.isfinite(d), np.isfinite(do))
+            ok = np.isfinite(do)
+            if ok.any():  # 1e-12 of the largest, and a few subnormal units where FP64 underflows term by term
+                assert np.max(np.abs(d[ok] - do[ok])) <= 1e-12 * np.max(np.abs(do[ok])) + 64 * 5e-324
