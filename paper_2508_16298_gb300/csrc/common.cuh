@@ -212,23 +212,34 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Sum over the first n lanes of a warp, valid in lane 0 (a block's last warp may be partial:
+// what a shuffle returns from a lane that is not there is not defined).
+__device__ __forceinline__ double lane_sum(double v, int n) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double t = __shfl_down_sync(0xffffffffu, v, o);
+    if (lane + o < n) v += t;
+  }
+  return v;
+}
+
 // Block sum of v; the result is valid in thread 0.  `scratch` holds >= 32 doubles.
 __device__ __forceinline__ double block_sum(double v, double* scratch) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  v = warp_sum(v);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = blockDim.x;
+  v = lane_sum(v, n - 32 * warp);
   __syncthreads();
   if (lane == 0) scratch[warp] = v;
   __syncthreads();
   double t = 0.0;
   if (warp == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-    t = (lane < nw) ? scratch[lane] : 0.0;
-    t = warp_sum(t);
+    const int nw = (n + 31) >> 5;
+    t = lane_sum((lane < nw) ? scratch[lane] : 0.0, nw);
   }
   return t;
 }
 
-// Sum of n partials by one warp in a fixed order; every lane returns the total.
+// Sum of n partials by one warp, all 32 lanes of it, in a fixed order; every lane returns the total.
 __device__ __forceinline__ double warp_sum_partials(const double* p, int n) {
   const int lane = threadIdx.x & 31;
   double s = 0.0;
@@ -237,7 +248,16 @@ __device__ __forceinline__ double warp_sum_partials(const double* p, int n) {
   return __shfl_sync(0xffffffffu, s, 0);
 }
 
-// The same sum with four running sums per lane (elements lane + 32 j, j mod 4):
+// The same by the one warp of a block of fewer than 32 threads.
+__device__ __forceinline__ double part_warp_sum_partials(const double* p, int n) {
+  const int lane = threadIdx.x, nl = blockDim.x;
+  double s = 0.0;
+  for (int k = lane; k < n; k += nl) s += p[k];
+  s = lane_sum(s, nl);
+  return __shfl_sync(0xffffffffu, s, 0);
+}
+
+// The same sum (a full warp) with four running sums per lane (elements lane + 32 j, j mod 4):
 // the dependent FP64 additions (slow on this part) form chains a quarter as
 // long, for a few more registers.  Used where hundreds of partials are summed
 // at the start of a kernel whose other registers dominate.

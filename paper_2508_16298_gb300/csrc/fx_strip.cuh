@@ -27,17 +27,6 @@ inline int fx_fraction_bits(double growth, double t) {
 __host__ __device__ inline int fx_nby(int L) { return L <= 50 ? 1 : 2; }
 __host__ __device__ inline int fx_threads(int L) { return L / 2 * ((L + 2 * fx_nby(L) - 1) / (2 * fx_nby(L))); }
 
-// Sum over the first n lanes of a warp, valid in lane 0 (a block's last warp may be partial).
-__device__ __forceinline__ double lane_sum(double v, int n) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const double t = __shfl_down_sync(0xffffffffu, v, o);
-    if (lane + o < n) v += t;
-  }
-  return v;
-}
-
 // W <- P W on a slice in shared memory, FP64, links converted from the table.
 static __device__ __noinline__ void slow_sweep(const Geo g, double2* W, const int4* __restrict__ U, const int nt) {
 #pragma unroll 1

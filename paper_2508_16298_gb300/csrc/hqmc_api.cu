@@ -1535,7 +1535,8 @@ int hqmc_make_config(const hqmc_params* p, hqmc_config** out) {
     cfg->sl32 = cfg->sl;
     cfg->sl32.mb = mb32;
     cfg->sl32.threads = th32;
-    // register-blocked variant: strips of nby 2x2 blocks, (L/2)^2/nby threads
+    // register-blocked variant: strips of nby 2x2 blocks, (L/2)^2/nby threads (a warp at least,
+    // except for the lowest strips of L <= 10, whose kernels have a head of their own)
     auto pick_block = [&](int real_bytes, SliceLaunch* out) {
       *out = cfg->sl;
       out->nby = 0;
@@ -1544,7 +1545,7 @@ int hqmc_make_config(const hqmc_params* p, hqmc_config** out) {
         if (Lh % nby) continue;
         const int th = Lh * Lh / nby;
         const int cap = block_thread_cap(real_bytes, nby);
-        if (cap <= 0 || th > cap) continue;
+        if (cap <= 0 || th > cap || (nby > 1 && th < 32)) continue;
         SliceLaunch c = cfg->sl;
         c.nby = nby;
         c.threads = th;
@@ -1573,6 +1574,7 @@ int hqmc_make_config(const hqmc_params* p, hqmc_config** out) {
       for (int nby = 1; nby <= 3; ++nby) {
         if (Lh % nby) continue;
         const int th = Lh * Lh / nby;
+        if (nby > 1 && th < 32) continue;  // as above
         if (th > walk_thread_cap(nby) || walk_smem_bytes(cfg->g, MODE_CGDIR) > prop.sharedMemPerBlockOptin) continue;
         SliceLaunch c = cfg->sl32;
         c.nby = nby;

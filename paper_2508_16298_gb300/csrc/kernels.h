@@ -109,8 +109,13 @@ struct MdagmArgs {
 // Partial sums of the head: four running sums per lane for the FP32 kernels (their
 // other registers dominate, and the dependent FP64 additions are slow); the compact
 // sum for the FP64 kernels, whose occupancy the extra registers would lower.
-template <class R>
+// SMALL: a strip kernel of fewer than 32 threads (L <= 10), whose warp lacks the lanes that
+// the other sums leave a share of the partials to.  An instantiation of its own: a call
+// in the head of every block costs the large lattices registers (46 -> 53 ms a trajectory
+// at L = 66).
+template <class R, bool SMALL>
 __device__ __forceinline__ double head_sum(const double* p, int n) {
+  if constexpr (SMALL) return part_warp_sum_partials(p, n);
   if constexpr (sizeof(R) == 4) return warp_sum_partials4(p, n);
   return warp_sum_partials(p, n);
 }
@@ -135,7 +140,7 @@ struct HeadAt {
   __device__ __forceinline__ const double* part_cross() const { return pcr; }
 };
 
-template <class R, class P>
+template <class R, bool SMALL, class P>
 __device__ __forceinline__ void cgdir_head_impl(const MdagmArgs<R>& a, const P& ptr, bool writer, int& s_flags,
                                                 R& s_beta, int& s_k) {
   if (threadIdx.x < 32) {
@@ -155,7 +160,7 @@ __device__ __forceinline__ void cgdir_head_impl(const MdagmArgs<R>& a, const P& 
     } else if (k == seg) {
       flags = 2;
       if (ptr.part_rz()) {
-        const double rz = head_sum<R>(ptr.part_rz(), a.n_part_rz);
+        const double rz = head_sum<R, SMALL>(ptr.part_rz(), a.n_part_rz);
         if (!isfinite(rz) || !(rz > 0.0)) {
           flags = 1;
           new_done = isfinite(rz) ? CG_BREAKDOWN : CG_NONFINITE;
@@ -164,10 +169,10 @@ __device__ __forceinline__ void cgdir_head_impl(const MdagmArgs<R>& a, const P& 
         }
       }
     } else {
-      const double rr = head_sum<R>(ptr.part_in(), a.n_part_in);
-      const double rz = ptr.part_rz() ? head_sum<R>(ptr.part_rz(), a.n_part_rz) : rr;
+      const double rr = head_sum<R, SMALL>(ptr.part_in(), a.n_part_in);
+      const double rz = ptr.part_rz() ? head_sum<R, SMALL>(ptr.part_rz(), a.n_part_rz) : rr;
       // flexible CG: beta = Re<z_k, r_k - r_{k-1}> / Re<z_{k-1}, r_{k-1}> (Polak-Ribiere)
-      const double cross = ptr.part_cross() ? head_sum<R>(ptr.part_cross(), a.n_part_rz) : 0.0;
+      const double cross = ptr.part_cross() ? head_sum<R, SMALL>(ptr.part_cross(), a.n_part_rz) : 0.0;
       if (!isfinite(rr) || !isfinite(rz) || !isfinite(cross)) {
         flags = 1;
         new_done = CG_NONFINITE;
@@ -202,18 +207,18 @@ __device__ __forceinline__ void cgdir_head_impl(const MdagmArgs<R>& a, const P& 
   __syncthreads();
 }
 
-template <class R>
+template <class R, bool SMALL = false>
 __device__ __forceinline__ void cgdir_head(const MdagmArgs<R>& a, bool writer, int& s_flags, R& s_beta,
                                            int& s_k) {
-  cgdir_head_impl<R>(a, HeadOwn<R>{a}, writer, s_flags, s_beta, s_k);
+  cgdir_head_impl<R, SMALL>(a, HeadOwn<R>{a}, writer, s_flags, s_beta, s_k);
 }
 
 // The head of one system of a multi-system launch (its state and partials given).
-template <class R>
+template <class R, bool SMALL = false>
 __device__ __forceinline__ void cgdir_head_at(const MdagmArgs<R>& a, bool writer, int& s_flags, R& s_beta,
                                               int& s_k, CgState* st, const double* part_in, const double* part_rz,
                                               const double* part_cross) {
-  cgdir_head_impl<R>(a, HeadAt{st, part_in, part_rz, part_cross}, writer, s_flags, s_beta, s_k);
+  cgdir_head_impl<R, SMALL>(a, HeadAt{st, part_in, part_rz, part_cross}, writer, s_flags, s_beta, s_k);
 }
 
 // Fused M^dagger M (three modes).

@@ -48,7 +48,8 @@ template <class R, int NBY> struct BlockThreads {
   static constexpr int max = sizeof(R) == 8 ? 640 : (NBY == 1 ? 1024 : (NBY == 2 ? 512 : 384));
 };
 
-template <class R, int MODE, int NBY>
+// SMALL (CGDIR, NBY = 1): a block of fewer than 32 threads (head_sum in kernels.h).
+template <class R, int MODE, int NBY, bool SMALL = false>
 __global__ void __launch_bounds__((BlockThreads<R, NBY>::max), 1) mdagm_block_kernel(const MdagmArgs<R> a) {
   pdl_begin();
   using T = C2<R>;
@@ -70,7 +71,7 @@ __global__ void __launch_bounds__((BlockThreads<R, NBY>::max), 1) mdagm_block_ke
   const bool active = tau < N;
 
   if (MODE == MODE_CGDIR) {
-    cgdir_head<R>(a, blockIdx.x == 0, s_flags, s_beta, s_k);
+    cgdir_head<R, SMALL>(a, blockIdx.x == 0, s_flags, s_beta, s_k);
     if (s_flags & 1) return;  // uniform over the whole grid: no cluster barrier is pending
   }
   const bool first = (MODE == MODE_CGDIR) && (s_flags & 2);
@@ -186,6 +187,9 @@ static cudaError_t block_launch(const SliceLaunch& sl, const MdagmArgs<R>& a, cu
   cfg.attrs = attr;
   attr[1] = pdl_attribute();
   cfg.numAttrs = 2;
+  if constexpr (MODE == MODE_CGDIR && NBY == 1) {
+    if (sl.threads < 32) return cudaLaunchKernelEx(&cfg, mdagm_block_kernel<R, MODE, NBY, true>, a);
+  }
   return cudaLaunchKernelEx(&cfg, mdagm_block_kernel<R, MODE, NBY>, a);
 }
 

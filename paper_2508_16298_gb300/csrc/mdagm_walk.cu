@@ -54,7 +54,8 @@ size_t walk_smem_bytes(const Geo& g, int mode, bool th64) {
 // TH64 (APPLY): theta is the field itself, in double; the angles are wrapped to float where the
 // links are formed, and the launch that would write the float table, and its reading
 // back, are saved.
-template <int MODE, int NBY, bool MULTI, bool TH64>
+// SMALL (CGDIR, NBY = 1): a block of fewer than 32 threads (head_sum in kernels.h).
+template <int MODE, int NBY, bool MULTI, bool TH64, bool SMALL = false>
 __global__ void __launch_bounds__(WalkThreads<NBY>::max, 1) mdagm_walk_kernel(const MdagmArgs<float> a,
                                                                                     const MultiStride ms) {
   pdl_begin();
@@ -136,7 +137,7 @@ __global__ void __launch_bounds__(WalkThreads<NBY>::max, 1) mdagm_walk_kernel(co
     }
   }
   if (MODE == MODE_CGDIR) {
-    cgdir_head_at<float>(a, rng == 0, s_flags, s_beta, s_k, st, a.part_in + poff,
+    cgdir_head_at<float, SMALL>(a, rng == 0, s_flags, s_beta, s_k, st, a.part_in + poff,
                          a.part_rz ? a.part_rz + poff : nullptr, a.part_cross ? a.part_cross + poff : nullptr);
     if (s_flags & 1) {  // uniform over the grid; the stage in flight lands before the block exits
       if (threadIdx.x == 0) mbar_wait_bounded(&bar, 0);
@@ -276,6 +277,9 @@ static cudaError_t walk_launch(const SliceLaunch& sl, const MdagmArgs<float>& a,
                                const MultiStride ms = MultiStride{1, 0, 0}) {
   const size_t smem = walk_smem_bytes(sl.g, MODE, TH64);
   const int grid = MULTI ? sl.grid * ms.nsys : sl.grid;
+  if constexpr (MODE == MODE_CGDIR && NBY == 1) {
+    if (sl.threads < 32) return launch_after(mdagm_walk_kernel<MODE, NBY, MULTI, TH64, true>, grid, sl.threads, smem, s, a, ms);
+  }
   return launch_after(mdagm_walk_kernel<MODE, NBY, MULTI, TH64>, grid, sl.threads, smem, s, a, ms);
 }
 
