@@ -24,7 +24,10 @@
 // partial sums (one slot per slice) too.
 //
 // A row that an infinity, a NaN or a non-finite angle reaches is computed in FP64
-// instead (slow_row), with the outcome FP64 arithmetic gives it.
+// instead (slow_row), with the outcome FP64 arithmetic gives it.  So is a row of an apply
+// that a slice of very uneven size enters (fx_uneven in fx.cuh): its small elements would
+// have fewer bits than a double.  A solve, which is judged by the norm of its residual,
+// has no such rows.
 #include "fx_strip.cuh"
 
 namespace hqmc {
@@ -42,7 +45,7 @@ size_t fx_smem_bytes(const Geo& g) {
   return (g.V + (fx_tmem(g.L) ? 2 : 1) * slot + 4 * fx_threads(g.L)) * sizeof(longlong2);
 }
 
-// ---- FP64 row for non-finite data ------------------------------------------------
+// ---- FP64 row for non-finite and uneven data ------------------------------------------------
 
 template <int MODE>
 __device__ __forceinline__ double2 fx_load(const MdagmArgs<double>& a, const double2* p_old, double beta, bool first,
@@ -126,6 +129,9 @@ __device__ __forceinline__ void fx_range(const MdagmArgs<double>& a, const int t
   __shared__ double s_beta;
   __shared__ int s_k;
   __shared__ uint32_t s_key[3];
+  // APPLY: of slice j in place j mod 8; set after its fetch, read after the second sweeps of the
+  // rows that use it, cleared four fetches ahead (a fetch's barrier lies between any two of these)
+  __shared__ int s_uneven[8];
   __shared__ double s_red[2][2][32];
   const int V = a.g.V, N = a.g.Ntau, L = a.g.L;
   longlong2* const E = reinterpret_cast<longlong2*>(smem_raw);
@@ -164,10 +170,10 @@ __device__ __forceinline__ void fx_range(const MdagmArgs<double>& a, const int t
   const int F = a.F;
   auto wrap = [N](int j) { return j < 0 ? j + N : (j >= N ? j - N : j); };
 
-  // Brings slice j (wrapped) into this thread's slots of X1 as doubles, writes p_new for
+  // Brings slice ju (mod N) into this thread's slots of X1 as doubles, writes p_new for
   // an own slice, and returns the slice's exponent (one barrier).
-  auto fetch = [&](int j, bool own, int slot) -> int {
-    const size_t base = (size_t)j * V;
+  auto fetch = [&](int ju, bool own, int slot) -> int {
+    const size_t base = (size_t)wrap(ju) * V;
     uint32_t key = 0;
 #pragma unroll
     for (int r = 0; r < H; ++r) {
@@ -182,10 +188,15 @@ __device__ __forceinline__ void fx_range(const MdagmArgs<double>& a, const int t
         key = max(key, max(fx_key(x.x), fx_key(x.y)));
       }
     }
+    const uint32_t strip = key;
     key = __reduce_max_sync(wmask, key);
     if (lane == 0) atomicMax(&s_key[slot], key);
-    if (tid == 0) s_key[slot == 2 ? 0 : slot + 1] = 0;  // of the next call: last read before the previous barriers
+    if (tid == 0) {  // of the next call: last read before the previous barriers
+      s_key[slot == 2 ? 0 : slot + 1] = 0;
+      if (MODE == MODE_APPLY) s_uneven[(ju + 4) & 7] = 0;
+    }
     __syncthreads();
+    if (MODE == MODE_APPLY && fx_uneven(strip, s_key[slot])) s_uneven[ju & 7] = 1;
     return fx_exponent(s_key[slot]);
   };
   // This thread's slots of X1 from doubles to fixed point.
@@ -212,10 +223,11 @@ __device__ __forceinline__ void fx_range(const MdagmArgs<double>& a, const int t
   };
 
   if (tid < 3) s_key[tid] = 0;
+  if (MODE == MODE_APPLY && tid < 8) s_uneven[tid] = 0;
   __syncthreads();
   longlong2 v[H][2], t[TREG ? H : 1][2];
   int e_prev = kFxZero;                                  // exponent of slice j - 1
-  int e_cur = fetch(wrap(tb - 1), false, 0);             // of slice j
+  int e_cur = fetch(tb - 1, false, 0);                   // of slice j
   int e_t = kFxZero, e_next = kFxZero, e_w = kFxZero;    // of t_j, slice j + 1, row j
   bool z_bad = true, zp_bad = true, slow = false;        // z_j, z_{j-1}, row j are not finite
   bool u_bad = links_bad(a, wrap(tb - 1));               // links of slice j
@@ -238,12 +250,13 @@ __device__ __forceinline__ void fx_range(const MdagmArgs<double>& a, const int t
     if (!second) {
       zp_bad = z_bad;
       z_bad = e_cur >= kFxBad || u_bad;
+      if (MODE == MODE_APPLY && j > tb) z_bad |= s_uneven[j & 7] != 0;  // barriers of row j - 1 lie between
     }
     if (second ? !slow : !z_bad) fx_sweep<NBY, AHEAD>(v, a.UF + (size_t)js * V * 2, sg, E, R0, R1);  // z_j, or P_j w_j
     if (!second) {
       const int jn = wrap(j + 1);
       u_bad = links_bad(a, jn);
-      e_next = fetch(jn, j + 1 < te, slot);
+      e_next = fetch(j + 1, j + 1 < te, slot);
       slot = slot == 2 ? 0 : slot + 1;
       if (j > tb && warp == 0 && MODE != MODE_APPLY) row_sums(j - 1);  // written before the barriers above
       const bool x_bad = e_next >= kFxBad;
@@ -285,6 +298,7 @@ __device__ __forceinline__ void fx_range(const MdagmArgs<double>& a, const int t
       if (own) continue;
     } else {
       double acc0 = 0.0, acc1 = 0.0;
+      if (MODE == MODE_APPLY && (s_uneven[(j - 1) & 7] | s_uneven[j & 7] | s_uneven[(j + 1) & 7])) slow = true;
       if (!slow) {
         const int n_t = e_w - e_t;
         // the row in fixed point to this thread's slots of X1's neighbour E (free since the
@@ -426,6 +440,7 @@ __device__ __forceinline__ void fx_apply_M_slice(const MdagmArgs<double>& a, int
   constexpr int H = 2 * NBY;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint32_t s_key;
+  __shared__ int s_uneven;
   const int V = a.g.V, N = a.g.Ntau, L = a.g.L;
   longlong2* const E = reinterpret_cast<longlong2*>(smem_raw);
   longlong2* const R0 = E + V;
@@ -439,7 +454,10 @@ __device__ __forceinline__ void fx_apply_M_slice(const MdagmArgs<double>& a, int
   const int4* const U = a.UF + (size_t)us * V * 2;
   const FxStrip sg = fx_strip<NBY>(L, tid);
   const bool full = NBY == 1 || sg.nr == H;
-  if (tid == 0) s_key = 0;
+  if (tid == 0) {
+    s_key = 0;
+    s_uneven = 0;
+  }
   __syncthreads();
   longlong2 v[H][2];
   uint32_t key = 0;
@@ -452,11 +470,25 @@ __device__ __forceinline__ void fx_apply_M_slice(const MdagmArgs<double>& a, int
       v[r][c] = make_longlong2(__double_as_longlong(x.x), __double_as_longlong(x.y));
       key = max(key, max(fx_key(x.x), fx_key(x.y)));
     }
+  const uint32_t strip = key;
   key = __reduce_max_sync(wmask, key);
   if (lane == 0) atomicMax(&s_key, key);
   __syncthreads();
   const int e = fx_exponent(s_key);
-  if (e >= kFxBad || links_bad(a, us)) {
+  bool fp64 = e >= kFxBad || links_bad(a, us);
+  if (!fp64) {
+    if (fx_uneven(strip, s_key)) s_uneven = 1;
+    const int s0 = fx_shift_base(e, a.F);
+#pragma unroll
+    for (int r = 0; r < H; ++r)
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        v[r][c] = make_longlong2(fx_from_double(__longlong_as_double(v[r][c].x), s0),
+                                 fx_from_double(__longlong_as_double(v[r][c].y), s0));
+    fx_sweep<NBY, NBY == 1>(v, U, sg, E, R0, R1);
+    fp64 = s_uneven != 0;  // set before the sweep's barriers
+  }
+  if (fp64) {
     double2* const W = reinterpret_cast<double2*>(E);
     for (int i = tid; i < V; i += nt) W[i] = a.x[bs + i];
     __syncthreads();
@@ -464,14 +496,6 @@ __device__ __forceinline__ void fx_apply_M_slice(const MdagmArgs<double>& a, int
     for (int i = tid; i < V; i += nt) a.y[bt + i] = caxpy(a.x[bt + i], f, W[i]);
     return;
   }
-  const int s0 = fx_shift_base(e, a.F);
-#pragma unroll
-  for (int r = 0; r < H; ++r)
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-      v[r][c] = make_longlong2(fx_from_double(__longlong_as_double(v[r][c].x), s0),
-                               fx_from_double(__longlong_as_double(v[r][c].y), s0));
-  fx_sweep<NBY, NBY == 1>(v, U, sg, E, R0, R1);
 #pragma unroll
   for (int r = 0; r < H; ++r)
 #pragma unroll

@@ -1,0 +1,75 @@
+"""Accuracy element by element of the operators a program can call, on vectors that are not of
+one size: point sources, sparse vectors and vectors that fall off over a slice.  The
+fixed-point kernels hold a slice to a fraction of its largest component, so slices
+like these take FP64 arithmetic.
+
+Bound: |y - y_oracle|_i <= c 2^-53 (A |x|)_i with A = |M|^T |M| or |M| of non-negative entries
+(theta = 0, all signs positive), the form of any FP64 evaluation's error.  A sweep is
+seven factors of four roundings each (two products, two additions, the link's own error
+among them), so M has 30 and M^dagger M 66 on either side: c = 150 covers both sides of
+both operators.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2508_16298_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+C = 150 * 2.0 ** -53
+
+
+@pytest.fixture(scope="module")
+def hq():
+    from paper_2508_16298_gb300 import build
+    build.build()
+    from paper_2508_16298_gb300 import hqmc
+    return hqmc
+
+
+def cuda(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def vectors(L, N):
+    """Sources by name: ones a slice, a few sites, a fall-off within every slice (below, at and far
+    beyond 2^-6 of its largest value, where the arithmetic changes), and one in tau."""
+    base = inputs.complex_gaussian(L, N, seed=202 + L)
+    g = inputs.rng(203 + L)
+    y, x = np.indices((L, L))
+    d = np.minimum(x, L - x) + np.minimum(y, L - y)
+    point = np.zeros_like(base)
+    point[N // 2, 3, L - 1] = 1.0
+    sparse = np.where(g.random(base.shape) < 0.01, base, 0)
+    out = {"point": point, "sparse": sparse, "two sizes": np.where(g.random(base.shape) < 0.5, base, base * 1e-12)}
+    for total in (3, 5, 6, 7, 9, 30, 300):  # binary orders over the slice
+        out["fall-off %d" % total] = base / np.abs(base) * 2.0 ** (-total * d / L)[None]
+    tau = out["fall-off 30"].copy()
+    for k in range(N):
+        tau[k] *= 10.0 ** (-7 * k)
+    out["fall-off in tau too"] = tau
+    return out
+
+
+def positive_M(lat, x, dagger):
+    """|M| |x|: apply_M at theta = 0 is x minus or plus B of the neighbour, B of positive entries."""
+    a = np.abs(x).astype(complex)
+    return a + np.abs(oracle.apply_M(lat, np.zeros((lat.Ntau, lat.L, lat.L, 2)), a, dagger=dagger) - a)
+
+
+@pytest.mark.parametrize("L,N", [(18, 6), (50, 3), (54, 4), (66, 3)])
+@pytest.mark.parametrize("start", ["zero", "hot"])
+def test_operators(hq, L, N, start):
+    lat = oracle.Lattice(L, N)
+    th = np.zeros((N, L, L, 2)) if start == "zero" else inputs.theta_hot(L, N, seed=201 + L)
+    with hq.Config(L, N) as cfg:
+        assert cfg.launch_shape(hq.FP64)["variant"] >= 200
+        for name, x in vectors(L, N).items():
+            for dagger in (False, True):
+                y = hq.apply_M(cfg, cuda(th), cuda(x), dagger=dagger).cpu().numpy()
+                bound = positive_M(lat, x, dagger).real
+                assert np.all(np.abs(y - oracle.apply_M(lat, th, x, dagger=dagger)) <= C * bound), (name, dagger)
+            y = hq.apply_MdagM(cfg, cuda(th), cuda(x)).cpu().numpy()
+            bound = positive_M(lat, positive_M(lat, x, False), True).real
+            assert np.all(np.abs(y - oracle.apply_MdagM(lat, th, x)) <= C * bound), name
