@@ -380,7 +380,8 @@ HQMC_API int hqmc_multi_launch_shape(const hqmc_config* cfg, int nrhs, int* rang
  * S_B the bosonic action (compact: (1/(J dtau)) sum[1 - cos(theta_{tau+1} -
  * theta_tau)], non-compact: (1/(J dtau)) sum (theta_{tau+1} - theta_tau)^2, plus
  * K dtau sum_plaquettes cos(curl theta)).  dSf (nullable) receives dS_f/dtheta
- * alone.  F and dSf are double[Ntau][L][L][2] and may not alias theta. */
+ * alone.  F and dSf are double[Ntau][L][L][2] and may not alias theta.  Accuracy: X's
+ * slices as in hqmc_apply_M. */
 HQMC_API int hqmc_force(hqmc_config* cfg, const double* theta, const void* X, double* F,
                double* dSf, void* stream);
 

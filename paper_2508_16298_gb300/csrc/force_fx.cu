@@ -71,7 +71,8 @@ __device__ __forceinline__ long long force_bond(longlong2& ui, longlong2& uj, lo
          fx_im(make_longlong2(wi.x - oi.x, wi.y - oi.y), ui, shift);
 }
 
-// The slice in FP64, for non-finite data.
+// The slice in FP64, for non-finite data and for slices of uneven size (fx_uneven), whose small
+// elements would have fewer bits than a double.
 struct LimbLinks {
   const int4* __restrict__ U;
   int L;
@@ -90,6 +91,7 @@ __device__ __forceinline__ void force_fx_slice(const MdagmArgs<double>& a, const
   constexpr int H = 2 * NBY;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint32_t s_key[2];
+  __shared__ int s_uneven;
   const int V = a.g.V, N = a.g.Ntau, L = a.g.L, Lh = L >> 1;
   longlong2* const E = reinterpret_cast<longlong2*>(smem_raw);
   longlong2* const R0 = E + V;
@@ -103,6 +105,7 @@ __device__ __forceinline__ void force_fx_slice(const MdagmArgs<double>& a, const
   const FxStrip s = fx_strip<NBY>(L, tid);
   const bool full = NBY == 1 || s.nr == H;
   if (tid < 2) s_key[tid] = 0;
+  if (tid == 0) s_uneven = 0;
   __syncthreads();
   // NBY = 2: w in this thread's slots of shared memory and dS_f summed in place, which the
   // 96 registers of a 4-row strip have no room for
@@ -127,6 +130,7 @@ __device__ __forceinline__ void force_fx_slice(const MdagmArgs<double>& a, const
       ku = max(ku, max(fx_key(x.x), fx_key(x.y)));
       kw = max(kw, max(fx_key(y.x), fx_key(y.y)));
     }
+  const uint32_t strip_u = ku, strip_w = kw;
   ku = __reduce_max_sync(wmask, ku);
   kw = __reduce_max_sync(wmask, kw);
   if (lane == 0) {
@@ -135,11 +139,9 @@ __device__ __forceinline__ void force_fx_slice(const MdagmArgs<double>& a, const
   }
   __syncthreads();
   const int eu = fx_exponent(s_key[0]), ew = max(eu, fx_exponent(s_key[1]));
-  if (ew >= kFxBad || links_bad(a, tau)) {
-    slow_force(a, fs, dSf, tau, smem_raw, nt);
-    return;
-  }
-  {
+  bool fp64 = ew >= kFxBad || links_bad(a, tau);
+  if (!fp64) {
+    if (fx_uneven(strip_u, s_key[0]) || fx_uneven(strip_w, s_key[1])) s_uneven = 1;
     const int s0 = fx_shift_base(eu, fs.Fu);
 #pragma unroll
     for (int r = 0; r < H; ++r)
@@ -147,8 +149,14 @@ __device__ __forceinline__ void force_fx_slice(const MdagmArgs<double>& a, const
       for (int c = 0; c < 2; ++c)
         u[r][c] = make_longlong2(fx_from_double(__longlong_as_double(u[r][c].x), s0),
                                  fx_from_double(__longlong_as_double(u[r][c].y), s0));
+    fx_sweep<NBY, NBY == 1>(u, U, s, E, R0, R1);  // P X_tau
+    fp64 = s_uneven != 0;  // set before the sweep's barriers
   }
-  fx_sweep<NBY, NBY == 1>(u, U, s, E, R0, R1);  // P X_tau
+  if (fp64) {
+    __syncthreads();  // the sweep's last reads of R1
+    slow_force(a, fs, dSf, tau, smem_raw, nt);
+    return;
+  }
   {  // w = Y_{tau+1} = X_{tau+1} - s cB P X_tau
     const int s0 = fx_shift_base(ew, fs.Fw), n = ew - eu + fs.Fu - fs.Fw;
     const bool plus = taup == 0;  // the antiperiodic wrap

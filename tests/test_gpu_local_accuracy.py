@@ -73,3 +73,26 @@ def test_operators(hq, L, N, start):
             y = hq.apply_MdagM(cfg, cuda(th), cuda(x)).cpu().numpy()
             bound = positive_M(lat, positive_M(lat, x, False), True).real
             assert np.all(np.abs(y - oracle.apply_MdagM(lat, th, x)) <= C * bound), name
+
+
+@pytest.mark.parametrize("L,N", [(18, 6), (50, 3), (54, 4), (66, 3)])
+def test_force(hq, L, N):
+    """dS_f of bond (i, j) is a product of u = P^-1 ... P X_tau and w = P ... Y_{tau+1}: the bound takes
+    each through non-negative B (theta = 0), and their errors together, 60 roundings of u, 40
+    of w and 5 of the product on either side: 210 2^-53."""
+    lat = oracle.Lattice(L, N)
+    th = inputs.theta_hot(L, N, seed=211 + L)
+    zero = np.zeros((L, L, 2))
+    t1 = np.tanh(lat.dtau * lat.t)
+    cB = np.cosh(lat.dtau * lat.t) * np.cosh(lat.dtau * lat.t / 2) ** 6
+    with hq.Config(L, N) as cfg:
+        for name, X in vectors(L, N).items():
+            d = torch.empty((N, L, L, 2), dtype=torch.float64, device="cuda")
+            hq.force(cfg, cuda(th), cuda(X), dSf=d)
+            a = np.abs(X).astype(complex)
+            b = np.stack([oracle.apply_B(lat, zero, v) for v in a])
+            u = np.stack([oracle.apply_B(lat, zero, v) for v in b]).real
+            w = np.stack([oracle.apply_B(lat, zero, v) for v in np.roll(a, -1, 0) + b]).real
+            bound = np.stack([w * np.roll(u, -1, ax) + np.roll(w, -1, ax) * u for ax in (2, 1)], axis=-1)
+            err = np.abs(d.cpu().numpy() - oracle.fermion_dS(lat, th, X))
+            assert np.all(err <= 210 * 2.0 ** -53 * 4 * t1 * cB * bound), name
