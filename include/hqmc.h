@@ -226,7 +226,10 @@ HQMC_API int hqmc_apply_MdagM(hqmc_config* cfg, const double* theta, const void*
  * which is Hermitian positive definite.
  *   r, z: device vectors (complex double for HQMC_FP64, complex float for HQMC_FP32),
  *   16-byte aligned, not overlapping.  The call uses config workspace (the FP64 or
- *   FP32 CG direction buffer) and is stream-ordered like every other call. */
+ *   FP32 CG direction buffer) and is stream-ordered like every other call.  FP64: a tile of
+ *   16 sites and some hundred slices is held in 64-bit fixed point where no eight of a site's
+ *   rows in it lie below 2^-4 of its largest component, else computed in FP64 arithmetic,
+ *   element by element; inside the solvers it is always in fixed point. */
 HQMC_API int hqmc_apply_precond(hqmc_config* cfg, const void* r, void* z, int precision, void* stream);
 
 /* The preconditioner's coefficients (host query): a, b, rho and W as above.  Any

@@ -131,7 +131,7 @@ HQMC_HD int fx_exponent(uint32_t key) {
 // (point sources, sparse or localised vectors) are computed in FP64 where a caller sees
 // the result itself.  Gaussian vectors, M^dagger of them and solutions on ordered and
 // on random fields (18^2 x 180 ... 66^2 x 660) stay above 2^-5.6.
-HQMC_HD bool fx_uneven(uint32_t strip, uint32_t key) { return strip + (6u << 20) < key; }
+HQMC_HD bool fx_uneven(uint32_t strip, uint32_t key, unsigned bits = 6) { return strip + (bits << 20) < key; }
 
 // Shift base of a slice of exponent E (an all-zero slice converts like the smallest one).
 HQMC_HD int fx_shift_base(int E, int F) { return 1085 - F + (E < -1021 ? -1021 : E); }

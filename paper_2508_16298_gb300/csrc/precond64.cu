@@ -10,7 +10,12 @@
 //
 // Growth: x = F_W u and F_W^dagger x each grow a component by at most 1/(1 - rho).  Where
 // a coefficient is out of the limbs' range (rho < 0.6), or a tile holds an infinity or a
-// NaN, the same passes run in FP64.
+// NaN, the same passes run in FP64.  So they do, in an application a program calls
+// (hqmc_apply_precond), for a tile in which some eight rows of a site lie below 2^-4 of the
+// largest component: the small elements of z would have fewer bits than a double there.
+// (Gaussian input, L = 48: error of z 7.5e-17 of its 2-norm at one scale, 1.7e-16 in FP64; at
+// 2^-4 the former is what FP64's rounding is on values so much smaller.)  CG is judged by
+// the norm of its residual.
 #include "fx_strip.cuh"
 #include "line_pos.cuh"
 
@@ -176,13 +181,14 @@ __device__ __forceinline__ double line_passes(const A& ar, const typename A::T* 
   return ar.total(xx);
 }
 
-// One tile: 16 sites (column bx), slices [t0, t1).
+// One tile: 16 sites (column bx), slices [t0, t1).  local: a tile of uneven size in FP64.
 __device__ __forceinline__ void line64_tile(const Geo& g, const LineCoef& lc, int t0, int t1,
                                             const double2* __restrict__ u, double2* __restrict__ z,
-                                            double* __restrict__ part, int bx, int slot) {
+                                            double* __restrict__ part, int bx, int slot, bool local) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32];
   __shared__ uint32_t s_key;
+  __shared__ int s_uneven;
   const int N = g.Ntau, V = g.V, W = lc.W;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = 2 * kSites * bx + lane;  // component of a slice
@@ -192,7 +198,10 @@ __device__ __forceinline__ void line64_tile(const Geo& g, const LineCoef& lc, in
   const size_t rowlen = 2 * (size_t)V;
   double* const U = reinterpret_cast<double*>(smem_raw);
   double* const X = U + (size_t)nu * 32;
-  if (threadIdx.x == 0) s_key = 0;
+  if (threadIdx.x == 0) {
+    s_key = 0;
+    s_uneven = 0;
+  }
   __syncthreads();
   // 1. the rows; every warp copies and converts every eighth
   const LinePos first = line_pos(t0 - W + warp, N);
@@ -212,8 +221,21 @@ __device__ __forceinline__ void line64_tile(const Geo& g, const LineCoef& lc, in
   key = __reduce_max_sync(0xffffffffu, key);
   if (lane == 0) atomicMax(&s_key, key);
   __syncthreads();
+  if (local) {  // uniform over the grid; each group of eight of this warp's rows (the last eight at the end)
+    const int nr = nu > warp ? (nu - warp + kWarps - 1) / kWarps : 0;
+    bool uneven = false;
+    for (int k = 0; k < nr; k += 8) {
+      const int k0 = max(0, min(k, nr - 8)), k1 = min(nr, k0 + 8);
+      uint32_t big = 0;
+      for (int m = k0; m < k1; ++m) big = max(big, fx_key(U[(warp + m * kWarps) * 32 + lane]));
+      big = max(big, __shfl_xor_sync(0xffffffffu, big, 1));  // of both components of the site
+      uneven |= fx_uneven(big, s_key, 4);
+    }
+    if (uneven) s_uneven = 1;
+    __syncthreads();
+  }
   int e = fx_exponent(s_key);
-  const bool fixed = lc.fx && e < kFxBad;
+  const bool fixed = lc.fx && e < kFxBad && !(local && s_uneven);
   // near the ends of the exponent range the rows are scaled on the way in and out
   const bool far = fixed && (e < -800 || e > 800);
   if (far) {
@@ -269,7 +291,8 @@ __global__ void __launch_bounds__(32 * kWarps, 3) line_precond64_kernel(Geo g, c
   pdl_begin();
   if (!line_gate(st)) return;  // uniform over the grid
   const int t0 = blockIdx.y * tc;
-  line64_tile(g, lc, t0, min(g.Ntau, t0 + tc), u, z, part, blockIdx.x, blockIdx.y * gridDim.x + blockIdx.x);
+  line64_tile(g, lc, t0, min(g.Ntau, t0 + tc), u, z, part, blockIdx.x, blockIdx.y * gridDim.x + blockIdx.x,
+              st == nullptr);
 }
 
 // Many chains in one launch: block b runs tile tiles[b] = (chain, bx, by) with that
@@ -283,7 +306,7 @@ __global__ void __launch_bounds__(32 * kWarps, 3) line_precond64_batch_kernel(
   __syncthreads();
   if (!line_gate(d.st)) return;  // uniform over the block
   const int t0 = t.z * d.tc;
-  line64_tile(d.g, d.lc, t0, min(d.g.Ntau, t0 + d.tc), d.u, d.z, d.part, t.y, t.z * d.gx + t.y);
+  line64_tile(d.g, d.lc, t0, min(d.g.Ntau, t0 + d.tc), d.u, d.z, d.part, t.y, t.z * d.gx + t.y, false);
 }
 
 }  // namespace

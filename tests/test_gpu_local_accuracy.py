@@ -96,3 +96,33 @@ def test_force(hq, L, N):
             bound = np.stack([w * np.roll(u, -1, ax) + np.roll(w, -1, ax) * u for ax in (2, 1)], axis=-1)
             err = np.abs(d.cpu().numpy() - oracle.fermion_dS(lat, th, X))
             assert np.all(err <= 210 * 2.0 ** -53 * 4 * t1 * cB * bound), name
+
+
+@pytest.mark.parametrize("L,N,dtau", [(18, 240, 0.1), (24, 131, 0.05), (10, 300, 0.2), (18, 20, 0.1)])
+def test_line_preconditioner(hq, L, N, dtau):
+    """Each pass is a sum over a site's line by a recursion acc <- v + rho acc: a rounding of one step
+    decays with rho, so the errors of x are those of |x| under the untruncated recursion G, and
+    z's those of both passes, scale G^T G^T G G |u|.  Three roundings a step here, W + 1 terms
+    summed one by one in the oracle: c = 2 (W + 1) + 16."""
+    from oracle import precond as opc
+    c = opc.coefficients(oracle.Lattice(L, N, dtau=dtau))
+
+    def recursion(v, back):
+        v = v[::-1] if back else v
+        acc, out = np.zeros_like(v[0]), np.empty_like(v)
+        for k in range(4 * N):  # until the start is forgotten: rho^(3 N) < 1e-9
+            acc = v[k % N] + c.rho * acc
+            out[k % N] = acc
+        return out[::-1] if back else out
+
+    along = inputs.complex_gaussian(L, N, seed=221)
+    k = np.arange(N)
+    lines = {"fall-off along tau %d" % s: along * 2.0 ** (-s * np.minimum(k, N - k) / N)[:, None, None] for s in (4, 40, 400)}
+    with hq.Config(L, N, dtau=dtau) as cfg:
+        for name, u in {**vectors(L, N), **lines, "real": along.real + 0j}.items():
+            z = hq.apply_precond(cfg, cuda(u)).cpu().numpy()
+            bound = np.abs(u)
+            for back in (False, False, True, True):
+                bound = recursion(bound, back)
+            tol = (2 * (c.W + 1) + 16) * 2.0 ** -53 * c.scale
+            assert np.all(np.abs(z - opc.apply(c, u)) <= tol * bound), name
