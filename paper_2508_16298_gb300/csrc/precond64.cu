@@ -236,6 +236,7 @@ __device__ __forceinline__ void line64_tile(const Geo& g, const LineCoef& lc, in
   }
   int e = fx_exponent(s_key);
   const bool fixed = lc.fx && e < kFxBad && !(local && s_uneven);
+  if (s_key == 0) e = 0;  // all zero: any scale
   // near the ends of the exponent range the rows are scaled on the way in and out
   const bool far = fixed && (e < -800 || e > 800);
   if (far) {
