@@ -110,7 +110,8 @@ typedef struct hqmc_params {
                               hqmc_make_config and keep the fastest; 0: built-in choice */
     int variant;           /* fused M^dagger M kernel: 0 any, 1 those of a batch (generic; FP64 in
                               fixed point from L = 12), 2 register-blocked
-                              only (HQMC_EUNSUPPORTED if no strip shape fits L), 3 FP32 on the
+                              only, in FP64 arithmetic where 0 and 1 are in fixed point
+                              (HQMC_EUNSUPPORTED if no strip shape fits L), 3 FP32 on the
                               persistent tau-walking kernel (HQMC_EUNSUPPORTED if it does not fit
                               L; FP64 as for 0) */
 } hqmc_params;
@@ -177,9 +178,9 @@ HQMC_API long long hqmc_launch_count(const hqmc_config* cfg);
 
 /* Launch shape of the fused M^dagger M for one precision (host query):
  * *variant >= 200: the fixed-point kernel of the FP64 operators with strips of
- * *variant - 200 2x2 blocks, one contiguous range of slices per CTA (every variant of
- * the parameters where L >= 18, variant 1 from L = 12, and tanh(dtau |t|) <= 0.3; the FP64
- * kernels below otherwise);
+ * *variant - 200 2x2 blocks, one contiguous range of slices per CTA (where L >= 18,
+ * variant 1 from L = 12, and tanh(dtau |t|) <= 0.3, but for variant 2; the FP64 kernels
+ * below otherwise);
  * 100 <= *variant < 200: persistent tau-walking kernel (FP32) with strips of
  * *variant - 100 2x2 blocks, one contiguous range of slices per CTA;
  * 0 < *variant < 100: register-blocked kernel with strips of *variant 2x2 blocks;
@@ -199,8 +200,8 @@ HQMC_API int hqmc_get_launch_shape(const hqmc_config* cfg, int precision, int* v
  * exponentials [[cosh a, e^{i theta} sinh a], [e^{-i theta} sinh a, cosh a]] with
  * a = dtau*t (halved for families 2-4).  precision: HQMC_FP64 (x, y complex
  * double) or HQMC_FP32 (complex float).  theta is always double.  x and y
- * must not overlap.  Accuracy in FP64: from L = 18 (variant 1: 12) and up to
- * tanh(dtau |t|) = 0.3 a slice is held in 64-bit fixed point, a unit being at most 2^-58 of
+ * must not overlap.  Accuracy in FP64: from L = 18 (variant 1: 12; variant 2: never) and
+ * up to tanh(dtau |t|) = 0.3 a slice is held in 64-bit fixed point, a unit being at most 2^-58 of
  * its largest component (errors of a few units), if each 2x2 block of its sites (4x2
  * above L = 50) has a component above 2^-6 of that; else, and on other lattices, in FP64
  * arithmetic, element by element. */

@@ -687,8 +687,8 @@ int enqueue_body(hqmc_config* cfg, int solver, const double2* phi, double2* x, c
   // the fused preconditioned update alternates two residual buffers, so an even
   // number of iterations per body leaves r where the body's residual expects it
   const bool fuse = pc && (iters % 2 == 0) && (mixed ? cfg->fuse_pc32 : cfg->fuse_pc64) && cfg->p.variant != 1;
-  // (timing wants an event per launch, variant 1 the batch's kernels)
-  const bool cluster = !mixed && !pc && cfg->cgc.ctas && cfg->p.variant != 1 && !cfg->timing;
+  // (timing wants an event per launch, variants 1 and 2 kernels of their own)
+  const bool cluster = !mixed && !pc && cfg->cgc.ctas && cfg->p.variant != 1 && cfg->p.variant != 2 && !cfg->timing;
   if (cluster) {
     MdagmArgs<double> a = mdagm_args<double, MODE_CGDIR>(cfg);
     a.U = cfg->U64;
@@ -1613,8 +1613,9 @@ int hqmc_make_config(const hqmc_params* p, hqmc_config** out) {
     // them, so rates count and not chains of products, and one launch for all of them beats
     // two (steps of 16 chains of L = 12 ... 24: 54.9 ms with FP64 below L = 18, 52.9 below 16,
     // 49.7 with none).  From L = 12 on a slice's block has a full warp, which the heads'
-    // sums need.  Variant 1, the batch's kernels for one chain, follows.
-    if (std::fabs(cfg->t1) <= kFxMaxLink && L >= (p->variant == 1 ? kFxMinBatchL : kFxMinL)) {
+    // sums need.  Variant 1, the batch's kernels for one chain, follows; variant 2 asks for
+    // the register-blocked FP64 kernel.
+    if (std::fabs(cfg->t1) <= kFxMaxLink && p->variant != 2 && L >= (p->variant == 1 ? kFxMinBatchL : kFxMinL)) {
       SliceLaunch f = cfg->sl;
       f.cluster = 1;
       f.mb = 0;

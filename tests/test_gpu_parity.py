@@ -419,3 +419,21 @@ def test_resume_from_checkpoint_is_bit_exact(hq, tmp_path):
                           dt=hdr["dt"], tol=1e-10)
     assert a["dH"] == b["dH"] and a["accepted"] == b["accepted"]
     assert torch.equal(th, th_b)
+
+
+@pytest.mark.parametrize("L,N", [(8, 13), (18, 5), (24, 33), (48, 7)])
+def test_register_blocked_variant_keeps_its_kernels(hq, L, N):
+    """variant 2 asks for the register-blocked kernels, in FP64 arithmetic, at every L they fit."""
+    lat = oracle.Lattice(L, N)
+    th, x = inputs.theta_hot(L, N, seed=221), inputs.complex_gaussian(L, N, seed=222)
+    for autotune in (False, True):
+        with hq.Config(L, N, variant=2, autotune=autotune) as cfg:
+            assert 0 < cfg.launch_shape(hq.FP64)["variant"] < 100 and 0 < cfg.launch_shape(hq.FP32)["variant"] < 100
+            assert rel(hq.apply_MdagM(cfg, cuda(th), cuda(x)).cpu().numpy(), oracle.apply_MdagM(lat, th, x)) < 1e-12
+            d = torch.empty((N, L, L, 2), dtype=torch.float64, device="cuda")
+            hq.force(cfg, cuda(th), cuda(x), dSf=d)
+            assert rel(d.cpu().numpy(), oracle.fermion_dS(lat, th, x)) < 1e-12
+            for solver in ("cg64", "pcg64", "mixed"):
+                X, i = hq.cg_solve(cfg, cuda(th), cuda(x), tol=1e-6, solver=solver)
+                res = x - oracle.apply_MdagM(lat, th, X.cpu().numpy())
+                assert i["status"] == 0 and np.linalg.norm(res) <= 1.01e-6 * np.linalg.norm(x)
