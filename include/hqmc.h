@@ -432,7 +432,8 @@ HQMC_API int hqmc_trajectory(hqmc_config* cfg, double* theta, uint64_t seed, uin
  * Ntau may differ; the batched kernels are the generic fused ones and every
  * chain gets the same cluster size, by default the smallest the chains admit).
  * If any params[c].autotune is set, hqmc_make_batch times the batched fused
- * launch at every cluster size 1, 2, 4, 8 the device co-schedules and every
+ * launch at cluster sizes 1, 2, 4, 8 the device co-schedules (chains on the FP64
+ * kernel), several numbers of slices per range (chains in fixed point) and every
  * tile order (hqmc_batch_launch_shape) and keeps the fastest; results do not
  * depend on that choice.  Each chain owns a config's workspace.  Inside a CG solve every iteration is ONE
  * launch of the fused M^dagger M over a tile table covering every chain's

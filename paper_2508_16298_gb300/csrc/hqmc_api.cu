@@ -2934,18 +2934,22 @@ cudaError_t batch_mdagm(hqmc_batch* b, const MdagmArgs<double>* descs, cudaStrea
 }
 
 // Autotuner of the batch: times the batched fused launch (an FP64 residual
-// r = phi - O x of every chain, Gaussian operands, links of theta = 0) at every
-// cluster size 1, 2, 4, 8 (and the same slices per range of the fixed-point chains) the
-// device can co-schedule and every tile order, and keeps the fastest.  Results do not depend on the choice: the neighbour's z_{tau-1}
-// is the same arithmetic as the recomputed halo, and the reduction slots are
-// per slice.
+// r = phi - O x of every chain, Gaussian operands, links of theta = 0) and keeps the fastest:
+// first every cluster size 1, 2, 4, 8 the device can co-schedule, where a chain is on the FP64
+// kernel, then the slices per range of the fixed-point chains, the model's choice
+// (batch_fx_range) and its neighbours among them, then the tile orders.  (Ranges tied to
+// the cluster sizes missed the model's: 3 chains of 48^2 x 480 took 512 us an iteration
+// with 2 slices a range instead of 428.)  Results do not depend on the choice: the
+// neighbour's z_{tau-1} is the same arithmetic as the recomputed halo, and the reduction
+// slots are per slice.
 int batch_autotune(hqmc_batch* b) {
   const int nc = (int)b->cfgs.size();
-  int minN = 1 << 30;
+  int minN = 1 << 30, maxFx = 0;  // shortest chain on the FP64 kernel, longest one in fixed point
   std::vector<MdagmArgs<double>> descs(nc);
   for (int c = 0; c < nc; ++c) {
     hqmc_config* cfg = b->cfgs[c];
-    minN = std::min(minN, cfg->p.Ntau);
+    if (chain_fx(cfg)) maxFx = std::max(maxFx, cfg->p.Ntau);
+    else minN = std::min(minN, cfg->p.Ntau);
     BCK(cudaMemset(cfg->th0, 0, 2 * cfg->n * sizeof(double)));
     for (int k = 0; k < 2; ++k) BCK(launch_draw_vector(cfg->n, 1, 3u, k, cfg->p64[k], cfg->bp.sintab, 0));
     b->launches += 2;
@@ -2970,31 +2974,43 @@ int batch_autotune(hqmc_batch* b) {
   float best = 1e30f;
   int bestC = b->C, bestR = b->fx_range, bestOrder = b->tile_order;
   int rc = HQMC_OK;
-  for (int C : {1, 2, 4, 8}) {
-    if (C > minN || (C > 1 && b->smem && mdagm_batch_max_active_clusters(C, b->threads, b->smem) <= 0)) continue;
-    for (int order = 0; order < 3 && rc == HQMC_OK; ++order) {
-      if ((rc = batch_set_tiles(b, C, C, order)) != HQMC_OK) break;
-      auto go = [&]() { return batch_mdagm<MODE_RESID>(b, b->d_resid_start, 0); };
-      cudaError_t err = go();
-      if (err == cudaSuccess) err = cudaEventRecord(e0, 0);
-      for (int k = 0; k < reps && err == cudaSuccess; ++k) err = go();
-      if (err == cudaSuccess) err = cudaEventRecord(e1, 0);
-      if (err == cudaSuccess) err = cudaEventSynchronize(e1);
-      float ms = 0.f;
-      if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
-      if (err != cudaSuccess) {  // a shape the device refuses is skipped
-        cudaGetLastError();
-        continue;
-      }
-      b->launches += (reps + 1) * b->n_mdagm;
-      const float us = 1e3f * ms / reps;
-      if (us < best) {
-        best = us;
-        bestC = bestR = C;
-        bestOrder = order;
-      }
+  auto time_tiles = [&](int C, int range, int order) {
+    if (rc != HQMC_OK || (rc = batch_set_tiles(b, C, range, order)) != HQMC_OK) return;
+    auto go = [&]() { return batch_mdagm<MODE_RESID>(b, b->d_resid_start, 0); };
+    cudaError_t err = go();
+    if (err == cudaSuccess) err = cudaEventRecord(e0, 0);
+    for (int k = 0; k < reps && err == cudaSuccess; ++k) err = go();
+    if (err == cudaSuccess) err = cudaEventRecord(e1, 0);
+    if (err == cudaSuccess) err = cudaEventSynchronize(e1);
+    float ms = 0.f;
+    if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
+    if (err != cudaSuccess) {  // a shape the device refuses is skipped
+      cudaGetLastError();
+      return;
     }
+    b->launches += (reps + 1) * b->n_mdagm;
+    const float us = 1e3f * ms / reps;
+    if (us < best) {
+      best = us;
+      bestC = C;
+      bestR = range;
+      bestOrder = order;
+    }
+  };
+  const int model = b->fx_range;
+  if (minN < 1 << 30) {
+    for (int C : {1, 2, 4, 8})
+      if (C <= minN && (C == 1 || mdagm_batch_max_active_clusters(C, b->threads, b->smem) > 0)) time_tiles(C, model, 0);
   }
+  if (maxFx) {
+    std::vector<int> ranges{1, 2, 4, 8, model / 2, model - 1, model, model + 1};
+    std::sort(ranges.begin(), ranges.end());
+    ranges.erase(std::unique(ranges.begin(), ranges.end()), ranges.end());
+    const int C = bestC;
+    for (int r : ranges)
+      if (r >= 1 && r <= maxFx) time_tiles(C, r, 0);
+  }
+  for (int order = 1; order < 3; ++order) time_tiles(bestC, bestR, order);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (rc != HQMC_OK) return rc;

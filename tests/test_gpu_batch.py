@@ -162,3 +162,22 @@ def test_batched_trajectory_against_oracle(hq, solver):
         assert bool(infos[i]["accepted"]) == ref["accepted"]
         want = ref["theta"] if ref["accepted"] else th0[i]
         assert np.max(np.abs(thetas[i].cpu().numpy() - want)) < 1e-8
+
+
+def test_autotuned_batch_is_not_slower_than_the_default(hq):
+    """Three chains of 48^2 x 480: the tuner's candidates hold the default's slices per range (ranges
+    of 1, 2, 4 or 8 alone cost 20 % here; runs of one shape differ by less than 2 %)."""
+    lat = [(48, 480)] * 3
+    ths = [torch.from_numpy(inputs.theta_ordered(L, N, 90 + i, tau_walk=0.0)).cuda() for i, (L, N) in enumerate(lat)]
+    phis = [torch.from_numpy(inputs.complex_gaussian(L, N, 95 + i)).cuda() for i, (L, N) in enumerate(lat)]
+    best = {}
+    for tune in (False, True):
+        with hq.Batch(lat, autotune=tune) as b:
+            for _ in range(5):
+                e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                e0.record()
+                b.cg_solve(ths, phis, tol=1e-14, maxit=160, raise_on_fail=False)
+                e1.record()
+                e1.synchronize()
+                best[tune] = min(best.get(tune, 1e9), e0.elapsed_time(e1))
+    assert best[True] <= 1.1 * best[False], best
