@@ -299,3 +299,46 @@ def test_force_at_the_ends_of_the_exponent_range(hq, L):
             ok = np.isfinite(do)
             if ok.any():  # 1e-12 of the largest, and a few subnormal units where FP64 underflows term by term
                 assert np.max(np.abs(d[ok] - do[ok])) <= 1e-12 * np.max(np.abs(do[ok])) + 64 * 5e-324
+
+
+@pytest.mark.parametrize("solver", ["cg64", "pcg64"])
+@pytest.mark.parametrize("autotune", [False, True])
+def test_batch_of_tall_strips_equals_single_chains(hq, solver, autotune):
+    """4-row strips in one batch: both block sizes (up to 512 threads and 608), two lattices of each,
+    whose blocks have idle rows (L mod 4 = 2) and surplus threads, several ranges a chain."""
+    lats = [(54, 8), (62, 6), (66, 5), (68, 4)]
+    th0 = [cuda(inputs.theta_ordered(L, N, 170 + i, tau_walk=0.0)) for i, (L, N) in enumerate(lats)]
+    phis = [cuda(inputs.complex_gaussian(L, N, 180 + i)) for i, (L, N) in enumerate(lats)]
+    with hq.Batch(lats, autotune=autotune) as b:
+        b.set_solver(solver)
+        xs, infos = b.cg_solve(th0, phis, tol=1e-10)
+        ths = [t.clone() for t in th0]
+        tinf = b.trajectory(ths, [5, 6, 7, 8], traj_counter=2, nsteps=2, dts=[0.005] * 4, tol=1e-9)
+    for i, (L, N) in enumerate(lats):
+        with hq.Config(L, N, variant=1) as cfg:
+            x1, info1 = hq.cg_solve(cfg, th0[i], phis[i], tol=1e-10, solver=solver)
+            t1 = th0[i].clone()
+            ti = hq.trajectory(cfg, t1, seed=5 + i, traj_counter=2, nsteps=2, dt=0.005, tol=1e-9, solver=solver)
+        assert infos[i]["status"] == 0 and infos[i]["iterations"] == info1["iterations"]
+        assert torch.equal(xs[i], x1) and infos[i]["true_residual"] == info1["true_residual"]
+        assert torch.equal(ths[i], t1) and tinf[i]["dH"] == ti["dH"] and tinf[i]["cg_iterations"] == ti["cg_iterations"]
+
+
+@pytest.mark.parametrize("L,N", [(20, 9), (54, 7), (66, 5)])
+@pytest.mark.parametrize("solver", ["mixed", "pmixed"])
+def test_multi_system_residuals_in_fixed_point(hq, L, N, solver):
+    """Systems solved together from L = 18: the FP64 residuals of every system, each range with its
+    own scratch, by the oracle's operator; solutions as starts are accepted as they are."""
+    lat, theta, nsys = oracle.Lattice(L, N), inputs.theta_ordered(L, N, 191, tau_walk=0.0), 3
+    phi = np.stack([inputs.complex_gaussian(L, N, 192 + k) * 10.0 ** (3 * k) for k in range(nsys)])
+    th = cuda(theta)
+    with hq.Config(L, N, reliable_interval=10) as cfg:
+        hq.set_multi_rhs(cfg, nsys)
+        X, infos = hq.cg_solve_multi(cfg, th, cuda(phi), tol=1e-9, solver=solver)
+        for k in range(nsys):
+            res = phi[k] - oracle.apply_MdagM(lat, theta, X[k].cpu().numpy())
+            true = np.linalg.norm(res) / np.linalg.norm(phi[k])
+            # the reported residual is that of x to the rounding of O x, a few 1e-16 |O| |x| / |phi|
+            assert infos[k]["status"] == 0 and abs(true - infos[k]["true_residual"]) < 1e-11 and true <= 1.01e-9
+        _, again = hq.cg_solve_multi(cfg, th, cuda(phi), x=X.clone(), tol=1e-9, solver=solver)
+        assert all(i["status"] == 0 and i["iterations"] == 0 for i in again)
