@@ -3424,7 +3424,7 @@ int hqmc_make_batch(const hqmc_params* params, int nchains, hqmc_batch** out) {
       const int nsb = ew(2 * cfg->n);  // the longest loop of the element-wise ops (2 per site)
       for (int j = 0; j < nsb; ++j) site_tab.push_back(make_int4(c, j, nsb, 0));
       for (int j = 0; j < cfg->act_grid; ++j) act_tab.push_back(make_int4(c, j, cfg->act_grid, 0));
-      const long long nff = (long long)cfg->g.V * ((cfg->p.Ntau + 7) / 8);  // one thread per site and 8 slices
+      const long long nff = (long long)cfg->g.V * ((cfg->p.Ntau + kFinishChunk - 1) / kFinishChunk);
       const int nfb = ew(nff);
       for (int j = 0; j < nfb; ++j) ff_tab.push_back(make_int4(c, j, nfb, 0));
       for (int t = 0; t < cfg->p.Ntau; ++t) {

@@ -527,7 +527,11 @@ struct BosonParams {
   int noncompact;
   const longlong2* sintab;  // 2^62 (cos, sin)(2 pi k / 256) (fx_sine_table); then the draws' logarithms
 };
-// F = -dSf - dS_B(theta).
+// F = -dSf - dS_B(theta), a thread for a site and kFinishChunk slices.  Eight: the term carried
+// from slice to slice saves 7 of 16 sines, and a small lattice still has the threads to hide
+// their latency.  With FP64 sines (bound by the FP64 rate) and chunks of 32 the kernel
+// took 316 us at L = 66, Ntau = 660 and 108 us at L = 24, Ntau = 240.
+constexpr int kFinishChunk = 8;
 cudaError_t launch_force_finish(const Geo& g, const BosonParams& bp, const double* theta,
                                 const double* dSf, double* F, cudaStream_t s);
 // p += h F

@@ -498,10 +498,6 @@ __device__ __forceinline__ double fprime(double d, const BosonParams& bp) {
 // the term f'(theta_{tau+1} - theta_tau) of slice tau is the f'(theta_tau' -
 // theta_{tau'-1}) of slice tau' = tau + 1, so it is evaluated once and carried
 // (the same operands in the same order: results identical to evaluating it twice).
-// Eight slices: the carried term saves 7 of 16 sines, and a small lattice still has the
-// threads to hide their latency.  With FP64 sines (bound by the FP64 rate) and chunks of
-// 32 this kernel took 316 us at L = 66, Ntau = 660 and 108 us at L = 24, Ntau = 240.
-constexpr int kFinishChunk = 8;
 
 __device__ __forceinline__ void force_finish_unit(const Geo& g, const BosonParams& bp, const double* __restrict__ theta,
                                                   const double* __restrict__ dSf, double* __restrict__ F, long long k);
