@@ -16,8 +16,8 @@
 //   here, passes in FP64                10.2     13.7       19.4    (576 threads: not used)
 //   here                                 9.4     13.3       14.8
 // (a trajectory of 11 solves at 8^2 x 40: 59.7 -> 29.8 ms; short solves count their start
-// here, so 6^2 is not below 8^2).  Up to 384 threads, one bond of each family for each: more
-// would not leave a thread its links in registers.
+// here, so 6^2 is not below 8^2).  Up to 384 threads, one bond of each family for each, in 154
+// to 162 registers; 576 threads, which 12^2 x 120 needs, would have 112 each (not measured).
 #include "fx_strip.cuh"
 #include "kernels.h"
 

@@ -50,9 +50,11 @@ size_t line_smem_bytes(int real_bytes, int W, int tc) { return (size_t)(tc + W +
 // 16 <= tc <= 256, with at least four tiles resident per SM and all tiles
 // resident at once (one round), ordered by the recursion work per SM (each
 // warp restarts both recursions W slices early: a fixed cost per tile); the
-// first is the default, the autotuner times them.  FP64 is bound by the FP64
-// FMA rate, so the work per slice decides: the tallest tc = ceil(N / k) <= 256
-// that still gives every SM two tiles, else 64.
+// first is the default, the autotuner times them.  FP64: the tallest tc = ceil(N / k)
+// <= 256 that still gives every SM two tiles of 32 sites, else 64, a rule found with
+// recursions in FP64, whose rate made the work per slice decide.  The fixed-point kernel
+// (precond64.cu), whose tiles are 16 sites wide, runs with the same heights; what others
+// take there is at line64_launch.
 std::vector<int> line_chunk_candidates(const Geo& g, int real_bytes, int W, int num_sms, size_t smem_per_sm) {
   std::vector<std::pair<double, int>> c;
   const long gx = (g.V + kLineSites - 1) / kLineSites;

@@ -49,7 +49,10 @@ void line_fx_coef(LineCoef& lc) {
   lc.fx = 1;
 }
 
-// Tiles: heights as line_chunk_candidates sets them.
+// Tiles: heights as line_chunk_candidates sets them (64, 96 at L = 48, 220 at L = 66).  One
+// application inside a solve, us, events around each launch, heights 64 / 96 / 165 / 220:
+// L = 24 14.3 / 15.8 / 18.4 / 20.4, L = 34 22.7 / 20.8 / 21.9 / 23.2, L = 48 45.0 / 36.8 / 35.0 /
+// 45.1, L = 66 100 / 82 / 81 / 105 (a tile of 220 slices fills an SM).
 LineLaunch line64_launch(const Geo& g, const LineCoef& lc, int num_sms, size_t smem_per_sm) {
   LineLaunch ll = line_launch(g, line_chunk_candidates(g, 8, lc.W, num_sms, smem_per_sm).front());
   while (ll.chunk > 16 && line64_smem_bytes(lc, ll.chunk) > std::min(smem_per_sm - 1024, kMaxSmem)) ll.chunk /= 2;
